@@ -234,7 +234,8 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMemcpy(d_w64, w64.data(), Ny * sizeof(double2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->flags, 0, FLAG_COUNT * sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, 2 * sizeof(unsigned), s);
-  if (e == cudaSuccess) e = plan_tc_power(p->sens, Nx, Nc, Ny, d_max, s);
+  const bool digits = p->storage == RECON_STORAGE_FP32 && plan_tc_admits(Ny);   // 16-bit: plan_tc.cu
+  if (e == cudaSuccess && digits) e = plan_tc_power(p->sens, Nx, Nc, Ny, d_max, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hmax, d_max, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->A, 0, (size_t)p->pk.col_elems * p->esize * ncols, s);
   if (e == cudaSuccess)
@@ -246,10 +247,10 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
   float power = 0.f, emax = 0.f;
   std::memcpy(&power, &hmax[0], sizeof(float));
   bool done = false;
-  if (e == cudaSuccess && plan_tc_admits(Ny) && 1.f + power / p->mu < kPlanTcMaxCond) {
+  if (e == cudaSuccess && digits && 1.f + power / p->mu < kPlanTcMaxCond) {
     if (cudaMalloc(&d_scr, plan_tc_scratch(Nx, Ny, Nt, p->num_sms)) == cudaSuccess) {
-      e = launch_plan_tc(p->sens, static_cast<double2*>(d_circ), p->mu, power, p->maxm, Nx, Ny, Nt, Nc, p->A, p->storage, p->pk,
-                         d_scr, d_max + 1, p->num_sms, p->flags, s);
+      e = launch_plan_tc(p->sens, static_cast<double2*>(d_circ), p->mu, power, p->maxm, Nx, Ny, Nt, Nc,
+                         static_cast<float2*>(p->A), p->pk, d_scr, d_max + 1, p->num_sms, p->flags, s);
       if (e == cudaSuccess) e = cudaMemcpyAsync(&hmax[1], d_max + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       std::memcpy(&emax, &hmax[1], sizeof(float));

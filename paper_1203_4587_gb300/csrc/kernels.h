@@ -502,7 +502,7 @@ cudaError_t launch_circulant(const int* rows, const int* rowoff, const double2* 
 cudaError_t launch_plan_inverse(const float2* sens, const double2* circ, double mu, int Nx, int Ny, int Nt, int Nc,
                                 void* A, int storage, const PackInfo& pk, double2* scratch, int grid,
                                 int* flags, cudaStream_t s);
-// Tensor-core inversion (plan_tc.cu), the same result for blocks whose
+// Tensor-core inversion (plan_tc.cu) of plans with FP32 storage, the same result for blocks whose
 // condition bound 1 + max sum_c |s|^2 / mu stays below kPlanTcMaxCond: the error
 // before the rounding grows with it and reaches about 2^-43 of max|A| there;
 // the double-float sweep takes 4 to 5 times as long at Ny = 128 and 256, but keeps
@@ -526,7 +526,7 @@ cudaError_t plan_tc_power(const float2* sens, int Nx, int Nc, int Ny, unsigned* 
 // plan_tc_max_e(1 + power / mu).  cudaErrorNotSupported: no tensor maps, nothing launched
 // maxm: the most sampled rows of a frame
 cudaError_t launch_plan_tc(const float2* sens, const double2* circ, float mu, float power, int maxm, int Nx, int Ny, int Nt, int Nc,
-                           void* A, int storage, const PackInfo& pk, void* scratch, unsigned* emax, int sms, int* flags,
+                           float2* A, const PackInfo& pk, void* scratch, unsigned* emax, int sms, int* flags,
                            cudaStream_t s);
 // The same for separate blocks (recon_gram_inverse_noalloc): mask [nblk][Ny], sens
 // [nblk][Nc][Ny], out [nblk][Ny][Ny] complex64, in the caller's scratch.
