@@ -254,7 +254,7 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
       if (e == cudaSuccess) e = cudaMemcpyAsync(&hmax[1], d_max + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       std::memcpy(&emax, &hmax[1], sizeof(float));
-      done = e == cudaSuccess && emax < 0.9375f * plan_tc_max_e(1.f + power / p->mu);
+      done = e == cudaSuccess && emax < 0.9375f * plan_tc_max_e(1.f + power / p->mu, Ny);
       if (e == cudaErrorNotSupported) e = cudaSuccess;
       cudaFree(d_scr);
       d_scr = nullptr;

@@ -504,18 +504,20 @@ cudaError_t launch_plan_inverse(const float2* sens, const double2* circ, double 
                                 int* flags, cudaStream_t s);
 // Tensor-core inversion (plan_tc.cu) of plans with FP32 storage, the same result for blocks whose
 // condition bound 1 + max sum_c |s|^2 / mu stays below kPlanTcMaxCond: the error
-// before the rounding grows with it and reaches about 2^-43 of max|A| there;
-// the double-float sweep takes 4 to 5 times as long at Ny = 128 and 256, but keeps
-// its accuracy.  At Ny = 64 (512 blocks) both take under a millisecond.
-constexpr int kPlanTcNyMax = 416;         // the sweep's panel and T in shared memory
+// before the rounding (plan_tc.cu) equals the double-float sweep's up to there, but grows with the square
+// of the condition where the sweep's grows with the condition;
+// the double-float sweep takes 4 to 5 times as long at Ny = 128 and 256.  At Ny = 64 (512
+// blocks) both take under a millisecond.
+constexpr int kPlanTcNyMax = 416;         // the largest size measured: accuracy, and exact digit sums
 constexpr float kPlanTcMaxCond = 64.f;
-// A power of two above max |E| of blocks of condition at most cond: |E| is about 2^-20.5
-// cond, so a factor of 2.8 to 5.7 is left.  Below 2^-13 (cond < 64) the error A E^3 stays
-// under 2^-40 of max|A|.
-inline float plan_tc_max_e(float cond) {
+// A power of two above max |E| of blocks of condition at most cond.  Measured over smooth and
+// random coils, 4 to 64 in condition, 50 to 416 in size: max |E| is up to 2^-23 (cond + 5) (Ny)^(1/4)
+// (the FP32 sweep's rounding, and X0's own 24 bits), and this lies 1.7 to 4 times above.  The digits
+// start there, so every bit of headroom costs one at the other end.
+inline float plan_tc_max_e(float cond, int Ny) {
   int e = 0;
-  std::frexp(cond, &e);
-  return std::ldexp(1.f, e - 19);
+  std::frexp((cond + 6.f) * std::sqrt(std::sqrt((float)Ny / 128.f)), &e);
+  return std::ldexp(1.f, e - 21);
 }
 inline int plan_tc_np(int Ny) { return (Ny + 31) / 32 * 32; }
 bool plan_tc_admits(int Ny);
@@ -523,7 +525,7 @@ size_t plan_tc_scratch(int Nx, int Ny, int Nt, int sms);
 // *out = max over (i, j) of sum_c |s_c|^2 as float bits (*out zeroed before; +inf for NaN or overflow)
 cudaError_t plan_tc_power(const float2* sens, int Nx, int Nc, int Ny, unsigned* out, cudaStream_t s);
 // A zeroed before; *emax receives max |E| as float bits: the caller checks it against 15/16 of
-// plan_tc_max_e(1 + power / mu).  cudaErrorNotSupported: no tensor maps, nothing launched
+// plan_tc_max_e(1 + power / mu, Ny).  cudaErrorNotSupported: no tensor maps, nothing launched
 // maxm: the most sampled rows of a frame
 cudaError_t launch_plan_tc(const float2* sens, const double2* circ, float mu, float power, int maxm, int Nx, int Ny, int Nt, int Nc,
                            float2* A, const PackInfo& pk, void* scratch, unsigned* emax, int sms, int* flags,
