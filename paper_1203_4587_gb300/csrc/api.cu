@@ -247,7 +247,7 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
   float power = 0.f, emax = 0.f;
   std::memcpy(&power, &hmax[0], sizeof(float));
   bool done = false;
-  if (e == cudaSuccess && digits && 1.f + power / p->mu < kPlanTcMaxCond) {
+  if (e == cudaSuccess && digits && plan_tc_conditioned(power, p->mu)) {
     if (cudaMalloc(&d_scr, plan_tc_scratch(Nx, Ny, Nt, p->num_sms)) == cudaSuccess) {
       e = launch_plan_tc(p->sens, static_cast<double2*>(d_circ), p->mu, power, p->maxm, Nx, Ny, Nt, Nc,
                          static_cast<float2*>(p->A), p->pk, d_scr, d_max + 1, p->num_sms, p->flags, s);

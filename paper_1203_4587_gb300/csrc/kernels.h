@@ -510,6 +510,12 @@ cudaError_t launch_plan_inverse(const float2* sens, const double2* circ, double 
 // blocks) both take under a millisecond.
 constexpr int kPlanTcNyMax = 416;         // the largest size measured: accuracy, and exact digit sums
 constexpr float kPlanTcMaxCond = 64.f;
+// power = max sum_c |s|^2.  The route scales M and A by powers of two in FP32, and the low halves of
+// the double-float products and the scaled c_t lose bits below 2^-126 (at mu = 1e-37 and 1e35 the
+// results were good to 2^-30 only): it takes mu between 2^-40 and 2^40, where nothing does.
+inline bool plan_tc_conditioned(float power, float mu) {
+  return 1.f + power / mu < kPlanTcMaxCond && mu > 9.0949470177e-13f && mu < 1.0995116278e12f;
+}
 // A power of two above max |E| of blocks of condition at most cond.  Measured over smooth and
 // random coils, 4 to 64 in condition, 50 to 416 in size: max |E| is up to 2^-23 (cond + 5) (Ny)^(1/4)
 // (the FP32 sweep's rounding, and X0's own 24 bits), and this lies 1.7 to 4 times above.  The digits

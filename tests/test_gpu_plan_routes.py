@@ -4,6 +4,7 @@
 import numpy as np
 import pytest
 
+import oracle
 import synthdata
 
 torch = pytest.importorskip("torch")
@@ -28,3 +29,20 @@ def test_16_bit_inverses_are_the_sweeps(storage):
     mask = synthdata.make_mask(256, 8, 6, np.random.default_rng(1))
     a = inverses(np.ascontiguousarray(sens[:, :, :64]), mask, 0.02, 64, storage=storage)   # bound 51
     assert torch.equal(a, inverses(sens, mask, 0.02, 64, storage=storage))
+
+
+# coils of 1e-18 and 1e18: products and their low halves reach the ends of the FP32 range
+@pytest.mark.parametrize("scale,mu", [(1e-18, 1e-37), (1e-9, 1e-18), (1e9, 1e17), (1e18, 1e35)])
+def test_blocks_far_from_one_in_scale(scale, mu):
+    """Half an FP32 ulp (a subnormal's at the least) plus 2^-41 max|A|, the bar at usual scales."""
+    from paper_1203_4587_gb300 import binding
+    sens = (scale * synthdata.make_sens(2, 72, 3, phase_y=0.3)).astype(np.complex64)
+    mask = synthdata.make_mask(72, 1, 3, np.random.default_rng(2))
+    cols = torch.from_numpy(np.ascontiguousarray(sens.transpose(2, 0, 1))).cuda()
+    A = binding.gram_inverse_noalloc(torch.from_numpy(np.repeat(mask, 2, axis=0).astype(np.uint8)).cuda(), cols, mu).cpu().numpy()
+    ref = oracle.inverse_blocks(oracle.gram_blocks(sens.astype(np.complex128), mask, [1])[0, 0], float(np.float32(mu)))
+    top = np.abs(ref).max()
+    for part in (np.real, np.imag):
+        a, r = part(A[1]).astype(np.float64), part(ref)
+        half = np.maximum(2.0 ** (np.floor(np.log2(np.maximum(np.abs(r), 1e-300))) - 24), 2.0 ** -150)
+        assert np.all(np.abs(a - r) <= half + 2.0 ** -41 * top)
