@@ -248,9 +248,16 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
   std::memcpy(&power, &hmax[0], sizeof(float));
   bool done = false;
   if (e == cudaSuccess && digits && plan_tc_conditioned(power, p->mu)) {
-    if (cudaMalloc(&d_scr, plan_tc_scratch(Nx, Ny, Nt, p->num_sms)) == cudaSuccess) {
+    // no room for a chunk: half of it, down to one image column; then the sweep
+    int cols = plan_tc_cols(Nx, Nt, p->num_sms, plan_tc_matrix_bytes(Ny), (double)p->pk.col_elems * p->esize * ncols);
+    while (cols > 0 && cudaMalloc(&d_scr, plan_tc_scratch(cols, Ny, Nt, p->num_sms)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      d_scr = nullptr;
+      cols /= 2;
+    }
+    if (cols > 0) {
       e = launch_plan_tc(p->sens, static_cast<double2*>(d_circ), p->mu, power, p->maxm, Nx, Ny, Nt, Nc,
-                         static_cast<float2*>(p->A), p->pk, d_scr, d_max + 1, p->num_sms, p->flags, s);
+                         static_cast<float2*>(p->A), p->pk, cols, d_scr, d_max + 1, p->num_sms, p->flags, s);
       if (e == cudaSuccess) e = cudaMemcpyAsync(&hmax[1], d_max + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       std::memcpy(&emax, &hmax[1], sizeof(float));
@@ -258,8 +265,6 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
       if (e == cudaErrorNotSupported) e = cudaSuccess;
       cudaFree(d_scr);
       d_scr = nullptr;
-    } else {
-      (void)cudaGetLastError();   // no room for the scratch: the sweep needs less
     }
   }
   if (e == cudaSuccess && !done) {

@@ -4,6 +4,7 @@
 //   fft_factor, fft_stages  the stage radices of the Stockham FFTs (every
 //                   transform of the library: rows, columns and time)
 //   lpt_work_lists  the per-CTA column lists of the column-inverse kernel
+//   plan_tc_cols    image columns that the tensor-core inversion takes at once
 //   mask_rows       the sampled ky rows of each frame of a Cartesian mask
 #pragma once
 
@@ -91,6 +92,16 @@ inline void lpt_work_lists(const std::vector<long long>& cost, const std::vector
     work_max = std::max(work_max, (int)per[b].size());
   }
   off[grid] = (int)work.size();
+}
+
+// Image columns (of Nt matrices each) a chunk of the tensor-core inversion: about 4 matrices an SM
+// (whole waves of every kernel), more while that is under 256 MB of scratch; but no more scratch
+// than 512 MB or the inverses it makes, whichever is more (a slab of 19 columns of 256 x 32 frames
+// makes 164 MB and would take 2.2 GB).
+inline int plan_tc_cols(int Nx, int Nt, int sms, double matrix_bytes, double inverse_bytes) {
+  const double most = std::max(536870912.0, inverse_bytes) / matrix_bytes;
+  const double mats = std::min(most, std::max(4.0 * sms, 2.56e8 / matrix_bytes));
+  return std::max(1, std::min(Nx, (int)(mats / Nt)));
 }
 
 // Sampled ky rows of a Cartesian ky-t mask (Section II-A: every kx of a

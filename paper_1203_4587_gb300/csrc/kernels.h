@@ -527,14 +527,15 @@ inline float plan_tc_max_e(float cond, int Ny) {
 }
 inline int plan_tc_np(int Ny) { return (Ny + 31) / 32 * 32; }
 bool plan_tc_admits(int Ny);
-size_t plan_tc_scratch(int Nx, int Ny, int Nt, int sms);
+double plan_tc_matrix_bytes(int Ny);   // scratch of one matrix
+size_t plan_tc_scratch(int cols, int Ny, int Nt, int sms);   // of a chunk of image columns (plan_tc_cols)
 // *out = max over (i, j) of sum_c |s_c|^2 as float bits (*out zeroed before; +inf for NaN or overflow)
 cudaError_t plan_tc_power(const float2* sens, int Nx, int Nc, int Ny, unsigned* out, cudaStream_t s);
 // A zeroed before; *emax receives max |E| as float bits: the caller checks it against 15/16 of
 // plan_tc_max_e(1 + power / mu, Ny).  cudaErrorNotSupported: no tensor maps, nothing launched
 // maxm: the most sampled rows of a frame
 cudaError_t launch_plan_tc(const float2* sens, const double2* circ, float mu, float power, int maxm, int Nx, int Ny, int Nt, int Nc,
-                           float2* A, const PackInfo& pk, void* scratch, unsigned* emax, int sms, int* flags,
+                           float2* A, const PackInfo& pk, int cols, void* scratch, unsigned* emax, int sms, int* flags,
                            cudaStream_t s);
 // The same for separate blocks (recon_gram_inverse_noalloc): mask [nblk][Ny], sens
 // [nblk][Nc][Ny], out [nblk][Ny][Ny] complex64, in the caller's scratch.
