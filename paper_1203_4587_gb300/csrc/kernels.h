@@ -539,6 +539,7 @@ cudaError_t launch_plan_tc(const float2* sens, const double2* circ, float mu, fl
                            cudaStream_t s);
 // The same for separate blocks (recon_gram_inverse_noalloc): mask [nblk][Ny], sens
 // [nblk][Nc][Ny], out [nblk][Ny][Ny] complex64, in the caller's scratch.
+cudaError_t block_tc_load();   // loads every kernel of the form onto the current device (lazy loading would at its first launch)
 int block_tc_chunk(int Ny, size_t bytes);   // blocks at once; 0: the scratch is too small
 // out[0] = power as plan_tc_power, out[1] = the most sampled rows of a block
 cudaError_t block_tc_bounds(const uint8_t* mask, const float2* sens, int Ny, int Nc, int nblk, unsigned* out, cudaStream_t s);
