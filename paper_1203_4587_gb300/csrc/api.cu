@@ -224,23 +224,26 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
     const double a = 2.0 * M_PI * (double)k / (double)Ny;
     w64[k] = make_double2(std::cos(a), std::sin(a));
   }
-  void *d_w64 = nullptr, *d_circ = nullptr, *d_scr = nullptr;
-  unsigned* d_max = nullptr;   // coil power, max |E|
+  void *d_tab = nullptr, *d_scr = nullptr;
   unsigned hmax[2] = {0, 0};
   const int grid = std::max(1, std::min<int>((int)ncols, p->num_sms));
-  cudaError_t e = cudaMalloc(&d_w64, Ny * sizeof(double2));
-  if (e == cudaSuccess) e = cudaMalloc(&d_circ, (size_t)Nt * Ny * sizeof(double2));
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&d_max), 2 * sizeof(unsigned));
+  cudaError_t e = cudaMalloc(&d_tab, (size_t)(Nt + 1) * Ny * sizeof(double2) + 2 * sizeof(unsigned));
+  auto* d_w64 = static_cast<double2*>(d_tab);
+  double2* d_circ = d_w64 + Ny;
+  auto* d_max = reinterpret_cast<unsigned*>(d_circ + (size_t)Nt * Ny);   // coil power, max |E|
   if (e == cudaSuccess) e = cudaMemcpy(d_w64, w64.data(), Ny * sizeof(double2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->flags, 0, FLAG_COUNT * sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, 2 * sizeof(unsigned), s);
-  const bool digits = p->storage == RECON_STORAGE_FP32 && plan_tc_admits(Ny);   // 16-bit: plan_tc.cu
-  if (e == cudaSuccess && digits) e = plan_tc_power(p->sens, Nx, Nc, Ny, d_max, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(hmax, d_max, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  const bool digits = p->storage == RECON_STORAGE_FP32 && plan_tc_admits(Ny) &&   // 16-bit: plan_tc.cu
+                      plan_tc_pays(Ny, (long long)ncols, p->num_sms);
+  if (e == cudaSuccess && digits) {
+    e = cudaMemsetAsync(d_max, 0, 2 * sizeof(unsigned), s);
+    if (e == cudaSuccess) e = plan_tc_power(p->sens, Nx, Nc, Ny, d_max, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hmax, d_max, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(p->A, 0, (size_t)p->pk.col_elems * p->esize * ncols, s);
   if (e == cudaSuccess)
-    e = launch_circulant(p->rows, p->rowoff, static_cast<double2*>(d_w64), static_cast<double2*>(d_circ), Ny, Nt, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    e = launch_circulant(p->rows, p->rowoff, d_w64, d_circ, Ny, Nt, s);
+  if (e == cudaSuccess && digits) e = cudaStreamSynchronize(s);
   // well-conditioned blocks on the tensor cores (G_{i,t} <= diag(sum_c |s|^2) bounds the
   // condition number); everything else, and a plan whose residual came out too
   // large, by the double-float sweep
@@ -256,7 +259,7 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
       cols /= 2;
     }
     if (cols > 0) {
-      e = launch_plan_tc(p->sens, static_cast<double2*>(d_circ), p->mu, power, p->maxm, Nx, Ny, Nt, Nc,
+      e = launch_plan_tc(p->sens, d_circ, p->mu, power, p->maxm, Nx, Ny, Nt, Nc,
                          static_cast<float2*>(p->A), p->pk, cols, d_scr, d_max + 1, p->num_sms, p->flags, s);
       if (e == cudaSuccess) e = cudaMemcpyAsync(&hmax[1], d_max + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -272,11 +275,11 @@ recon_status plan_invert(recon_plan* p, cudaStream_t s) {
     // triangles of all CTAs then stay in L2 up to Ny = 256
     e = cudaMalloc(&d_scr, (size_t)grid * Ny * Ny * sizeof(double2));
     if (e == cudaSuccess)
-      e = launch_plan_inverse(p->sens, static_cast<double2*>(d_circ), (double)p->mu, Nx, Ny, Nt, Nc, p->A, p->storage,
+      e = launch_plan_inverse(p->sens, d_circ, (double)p->mu, Nx, Ny, Nt, Nc, p->A, p->storage,
                               p->pk, static_cast<double2*>(d_scr), grid, p->flags, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  cudaFree(d_w64); cudaFree(d_circ); cudaFree(d_scr); cudaFree(d_max);
+  cudaFree(d_tab); cudaFree(d_scr);
   if (e != cudaSuccess) return cuda_fail(e, "plan inverse");
   int fl[FLAG_COUNT];
   RC(cudaMemcpy(fl, p->flags, sizeof(fl), cudaMemcpyDeviceToHost));

@@ -4,7 +4,8 @@
 //   fft_factor, fft_stages  the stage radices of the Stockham FFTs (every
 //                   transform of the library: rows, columns and time)
 //   lpt_work_lists  the per-CTA column lists of the column-inverse kernel
-//   plan_tc_cols    image columns that the tensor-core inversion takes at once
+//   plan_tc_cols    image columns that the tensor-core inversion takes at once;
+//   plan_tc_pays, block_tc_pays  the sizes from which it takes less time than the other forms
 //   mask_rows       the sampled ky rows of each frame of a Cartesian mask
 #pragma once
 
@@ -102,6 +103,36 @@ inline int plan_tc_cols(int Nx, int Nt, int sms, double matrix_bytes, double inv
   const double most = std::max(536870912.0, inverse_bytes) / matrix_bytes;
   const double mats = std::min(most, std::max(4.0 * sms, 2.56e8 / matrix_bytes));
   return std::max(1, std::min(Nx, (int)(mats / Nt)));
+}
+
+// Whether the tensor-core inversion pays for a plan of mats = Nx Nt blocks: its dozen launches, scratch
+// allocation and second synchronisation cost 100 to 300 us, which small sizes only earn with many
+// blocks.  recon_plan_set_mu, double-float sweep and this, us (152 SMs):
+//   Ny = 48    64 blocks 387 / 467, 608 647 / 728, 2432 1596 / 1692: never
+//   Ny = 56   304 blocks 541 / 584, 608 784 / 723, 2432 2100 / 1695: four blocks an SM
+//   Ny = 64    16 blocks 275 / 445, 152 448 / 490, 304 595 / 571, 608 872 / 725: two an SM
+//   Ny = 80     4 blocks 376 / 472, 16 536 / 491, 152 588 / 588, 608 1320 / 1040: 16
+//   Ny = 96     4 blocks 515 / 474, 152 724 / 584, 2432 6351 / 2603: always
+inline bool plan_tc_pays(int Ny, long long mats, int sms) {
+  if (Ny >= 96) return true;
+  if (Ny >= 80) return mats >= 16;
+  return Ny >= 56 && mats >= (Ny >= 64 ? 2ll : 4ll) * sms;
+}
+
+// The same for nblk separate blocks that run `chunk` at a time (a chunk of 16 MiB costs 115 us up to
+// Ny = 64 and 150 to 96, whatever its blocks' own size), against as many FP64 workspaces as there is
+// room for.  FP64 and this, us:
+//   Ny = 33    70 blocks 286 / 172, 130 279 / 290, 1024 844 / 1716: one chunk
+//   Ny = 40   130 blocks 379 / 288, 256 460 / 513: two
+//   Ny = 44   130 blocks 432 / 288, 512 790 / 951: three
+//   Ny = 48   130 blocks 484 / 288, 2048 3305 / 3247: any
+//   Ny = 65   256 blocks 1809 / 1271, 512 2803 / 2456, 1024 4794 / 4826, 2048 8740 / 9617: 20 chunks
+//   Ny = 72  2048 blocks 13362 / 9692: any
+inline bool block_tc_pays(int Ny, int nblk, int chunk) {
+  if (Ny < 33 || chunk < 1) return false;
+  const int chunks = (nblk - 1) / chunk + 1;
+  if (Ny < 48) return chunks <= (Ny >= 44 ? 3 : Ny >= 36 ? 2 : 1);
+  return Ny < 65 || Ny >= 70 || chunks <= 20;
 }
 
 // Sampled ky rows of a Cartesian ky-t mask (Section II-A: every kx of a

@@ -541,7 +541,7 @@ cudaError_t launch_plan_tc(const float2* sens, const double2* circ, float mu, fl
 // [nblk][Nc][Ny], out [nblk][Ny][Ny] complex64, in the caller's scratch.
 cudaError_t block_tc_load();   // loads every kernel of the form onto the current device (lazy loading would at its first launch)
 int block_tc_chunk(int Ny, size_t bytes);   // blocks at once; 0: the scratch is too small
-// out[0] = power as plan_tc_power, out[1] = the most sampled rows of a block
+// out[0] = power as plan_tc_power, out[1] = the most sampled rows of a block (both zeroed before)
 cudaError_t block_tc_bounds(const uint8_t* mask, const float2* sens, int Ny, int Nc, int nblk, unsigned* out, cudaStream_t s);
 cudaError_t launch_block_tc(const uint8_t* mask, const float2* sens, float mu, float power, int maxm, int Ny, int Nc, int nblk,
                             float2* out, void* scratch, size_t bytes, unsigned* emax, int sms, int* flags, cudaStream_t s);

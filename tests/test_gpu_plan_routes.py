@@ -46,3 +46,46 @@ def test_blocks_far_from_one_in_scale(scale, mu):
         a, r = part(A[1]).astype(np.float64), part(ref)
         half = np.maximum(2.0 ** (np.floor(np.log2(np.maximum(np.abs(r), 1e-300))) - 24), 2.0 ** -150)
         assert np.all(np.abs(a - r) <= half + 2.0 ** -41 * top)
+
+
+def launches(call):
+    from paper_1203_4587_gb300 import binding
+    n = binding.kernel_launches()
+    call()
+    return binding.kernel_launches() - n
+
+
+# on 152 SMs: 96 and above always, 80 with 16 blocks, 64 with two blocks an SM, 56 with four, never below;
+# 416 is the largest size (csrc/host_logic.h)
+@pytest.mark.parametrize("Ny,Nx,Nt,tensor", [(48, 160, 8, False), (55, 160, 8, False), (56, 75, 8, False), (56, 76, 8, True),
+                                             (64, 37, 8, False), (64, 38, 8, True), (80, 3, 5, False), (80, 2, 8, True),
+                                             (96, 1, 1, True), (416, 1, 1, True), (417, 1, 1, False)])
+def test_plan_route_by_size(Ny, Nx, Nt, tensor):
+    """Small plans are not slower for the tensor cores' launches: the sweep is two kernels (three with the
+    condition's bound), the tensor-core form five a chunk and three more."""
+    from paper_1203_4587_gb300 import Plan
+    sens = synthdata.make_sens(Nx, Ny, 2, phase_y=0.3).astype(np.complex64)
+    mask = synthdata.make_mask(Ny, Nt, 3, np.random.default_rng(Ny))
+    P = Plan(mask.astype(np.uint8), torch.from_numpy(sens).cuda(), 0.01, 0.1, max_iters=1)
+    n = launches(lambda: P.set_mu(0.1))
+    assert n >= 8 if tensor else n <= 3
+    P.close()
+
+
+# a chunk of 16 MiB holds 72 blocks up to 64, 32 up to 96
+@pytest.mark.parametrize("Ny,nblk,tensor", [(32, 1, False), (33, 60, True), (33, 130, False), (36, 130, True), (40, 256, False),
+                                            (44, 200, True), (44, 512, False), (48, 1024, True), (65, 256, True),
+                                            (65, 1024, False), (72, 1024, True)])
+def test_blocks_route_by_size(Ny, nblk, tensor):
+    from paper_1203_4587_gb300 import binding
+    sens = torch.full((nblk, 2, Ny), 0.7, dtype=torch.complex64, device="cuda")
+    mask = (torch.arange(Ny, device="cuda") % 3 == 0).to(torch.uint8).repeat(nblk, 1)
+    n = launches(lambda: binding.gram_inverse_noalloc(mask, sens, 0.1))
+    assert n >= 8 if tensor else n <= 3
+
+
+@pytest.mark.parametrize("Ny", [56, 63, 64, 65, 72, 80, 95])
+def test_small_sizes_on_the_tensor_cores(Ny):
+    """Enough blocks for the tensor-core form below 96: tile edges and padding, as test_gpu_plan_tc.py."""
+    from test_gpu_plan_tc import check
+    check(Ny, 0.1, Nx=77, Nt=8)
