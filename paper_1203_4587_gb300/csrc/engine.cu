@@ -423,7 +423,7 @@ int engine_default_tile(const Engine* e) {
   if (e->prior == RECON_PRIOR_HAAR) return haar_tile_px(e->Nt_max, e->levels);
   long long pixels = 0;
   for (recon_plan* p : e->plans) pixels += (long long)p->npix();
-  return dft_tile_px(pixels, e->plans[0]->num_sms);
+  return dft_tile_px(pixels, e->plans[0]->num_sms, e->Nt_max);
 }
 
 // (Re)builds the K+1 temporal descriptor sets for tiles of `px` pixels.

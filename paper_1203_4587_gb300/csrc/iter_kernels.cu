@@ -572,10 +572,11 @@ cudaError_t launch_tv_temporal(const TemporalLaunch& p, cudaStream_t s, bool pdl
 // accumulates ||w||_1 (the prior term of J at the incoming iterate).
 // ---------------------------------------------------------------------------
 static size_t dft_smem(int Nt_max, int px) { return 2 * (size_t)Nt_max * px * sizeof(float2); }
-// Default tile: 32 pixels where 64 would leave fewer than four blocks an SM (a
-// block is one chain of dependent stages).  200 iterations at 128 x 128 x 22:
-// 16 px 12.8 ms, 32 px 10.75, 64 px 11.0, 128 px 12.0.
-int dft_tile_px(long long pixels, int sms) { return pixels / 64 < 4ll * sms ? 32 : 64; }
+// Default tile: 32 pixels where all such blocks are resident at once (four an SM) and there are frames
+// enough to fill 256 threads; a block is one chain of dependent stages, and more of them hide it.
+// 40 iterations, 64 and 32 pixels, us: 96 x 96 x 16 1311 / 1257, 128 x 128 x 22 2331 / 2242; beyond, 160 x
+// 160 x 8 1580 / 1798 and 192 x 192 x 16 3528 / 3748; with few frames, 128 x 128 x 3 764 / 801.
+int dft_tile_px(long long pixels, int sms, int Nt) { return Nt > 4 && pixels <= 128ll * sms ? 32 : 64; }
 int dft_tile_candidates(int Nt_max, int* out) {
   int n = 0;
   for (int px : {16, 32, 64, 128})

@@ -422,7 +422,7 @@ cudaError_t prepare_tv_temporal(int Nt_max, int px);   // shared-memory attribut
 cudaError_t prepare_dft_temporal(int Nt_max, int px);
 cudaError_t prepare_col_inverse(int storage, size_t smem);
 int tv_tile_px(int Nt_max);                         // default pixels per block
-int dft_tile_px(long long pixels, int sms);      // pixels of all slices of a launch
+int dft_tile_px(long long pixels, int sms, int Nt);   // pixels of all slices of a launch, its most frames
 int tv_tile_candidates(int Nt_max, int* out);       // tile widths that fit (<= 4 entries)
 int dft_tile_candidates(int Nt_max, int* out);
 cudaError_t launch_tv_temporal(const TemporalLaunch& p, cudaStream_t s, bool pdl = false);
