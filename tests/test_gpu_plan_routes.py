@@ -89,3 +89,27 @@ def test_small_sizes_on_the_tensor_cores(Ny):
     """Enough blocks for the tensor-core form below 96: tile edges and padding, as test_gpu_plan_tc.py."""
     from test_gpu_plan_tc import check
     check(Ny, 0.1, Nx=77, Nt=8)
+
+
+def test_ill_conditioned_and_non_finite_blocks_of_the_tensor_cores_sizes():
+    """Two kernels for the bounds and the FP64 one; a well-conditioned call afterwards takes the six of the
+    tensor cores."""
+    from paper_1203_4587_gb300 import binding
+    lib = binding.load()
+    Ny = 40
+    sens = synthdata.make_sens(3, Ny, 3, phase_y=0.3).astype(np.complex64)
+    mask = synthdata.make_mask(Ny, 1, 3, np.random.default_rng(4))
+    m = torch.from_numpy(np.repeat(mask, 3, axis=0).astype(np.uint8)).cuda()
+    cols = torch.from_numpy(np.ascontiguousarray(sens.transpose(2, 0, 1))).cuda()
+    for mu in (0.005, 0.1):
+        A = binding.gram_inverse_noalloc(m, cols, mu).cpu().numpy()
+        assert launches(lambda: binding.gram_inverse_noalloc(m, cols, mu)) == (3 if mu < 0.01 else 8)
+        ref = oracle.inverse_blocks(oracle.gram_blocks(sens.astype(np.complex128), mask, [2])[0, 0], float(np.float32(mu)))
+        top = np.abs(ref).max()
+        for part in (np.real, np.imag):
+            a, r = part(A[2]).astype(np.float64), part(ref)
+            assert np.all(np.abs(a - r) <= 0.5 * np.spacing(np.abs(r).astype(np.float32)) + 2.0 ** -41 * top)
+    bad = cols.clone()
+    bad[1, 0, 3] = complex(float("inf"), 0.0)
+    out = torch.empty((3, Ny, Ny), dtype=torch.complex64, device="cuda")
+    assert lib.recon_gram_inverse_noalloc(Ny, 3, 3, binding._ptr(m), binding._ptr(bad), 0.1, binding._ptr(out), None) == 6
