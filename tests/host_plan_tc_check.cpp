@@ -11,7 +11,7 @@ int main() {
       for (int nx : widths) {
         const double np = (ny + 31) / 32 * 32, per = 56.0 * np * np, inv = 4.0 * np * np * nx * nt;
         const int c = recon::plan_tc_cols(nx, nt, 152, per, inv);
-        const double got = c * nt * per, most = inv > 536870912.0 ? inv : 536870912.0;
+        const double got = c * nt * per, most = 1.25 * inv > 6e8 ? 1.25 * inv : 6e8;
         bool ok = c >= 1 && c <= nx;
         ok = ok && (c == 1 || got <= most);                             // the stated limit on the scratch
         const double want = 608 * per > 2.56e8 ? 608 * per : 2.56e8;   // and no less than it allows

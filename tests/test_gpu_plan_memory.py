@@ -44,7 +44,7 @@ def ends(P, Nx, Nt):
     return torch.stack([P.export_inverse(i, t) for i in (0, Nx // 2, Nx - 1) for t in (0, Nt - 1)])
 
 
-# 64 columns of 16 frames, 128 x 128: chunks of 36 columns (528 MB) as they come, 8 or 9 in 150 MB
+# 64 columns of 16 frames, 128 x 128: chunks of 38 columns (558 MB) as they come, 8 or 9 in 150 MB
 @pytest.mark.parametrize("Nx,Ny,Nt,free_mb,chunks", [(64, 128, 16, 150, True), (8, 64, 128, 24, False)])
 def test_set_mu_with_little_memory(Nx, Ny, Nt, free_mb, chunks):
     """(8 columns of 128 frames of 64 x 64: one column takes 38 MB, the sweep 10 MB.)"""

@@ -1,5 +1,5 @@
 """The chunk rule of the tensor-core inversion on the CPU (paper_1203_4587_gb300/csrc/host_logic.h):
-at least one image column, never more scratch than 512 MB or the inverses it makes, and no less than
+at least one image column, never more scratch than 600 MB or a quarter more than the inverses it makes, and no less than
 that allows."""
 
 import os
