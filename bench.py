@@ -627,11 +627,12 @@ def measure_grad(storage, steps=5):
         p.close()
     f, b = statistics.median(fwd), statistics.median(bwd)
     # algorithmic bytes: the packed inverses (the Hermitian triangle of every
-    # column) streamed once per inverse launch: K forward steps; K reverse
-    # steps plus K - K/every recomputed steps backward
+    # column) streamed once per inverse launch: K forward steps; K reverse steps
+    # backward, plus the inner steps of every segment but the last, which the
+    # forward leaves in place
     Nt, Ny, Nx = cases[0].x_true.shape
     a_bytes = len(cases) * (8 if storage == "fp32" else 4) * Nx * Nt * Ny * (Ny + 1) // 2
-    n_fwd, n_bwd = iters, iters + (iters - iters // every)
+    n_fwd, n_bwd = iters, iters + ((iters - 1) // every) * (every - 1)
     peak, _ = hbm_peak()
     fgbs = n_fwd * a_bytes / (f / 1e3) / 1e9
     bgbs = n_bwd * a_bytes / (b / 1e3) / 1e9
